@@ -104,18 +104,24 @@ struct FrItem {
   int32_t j0, n;       // range in the job's brick-ordered column list
 };
 
-// Byte offsets of one warp's shared-memory arena.
+// One warp's shared-memory arena.  The sections whose size does not depend on
+// the launch lie at fixed offsets, so that a function which only gets the
+// arena's offset reaches them (and the family matrices after them) with
+// constant addresses:
+//   header (the voxel's window, VoxHdr), lut (level -> compact index), lev
+//   (compact index -> level), st (start of each level run in the sorted keys),
+//   fv (features), acc (per-direction accumulators), tmp, big (family
+//   matrices, layout from (mc, bc, w)), then kb (sort keys / zone keys) and
+//   lvl (compact level + 1 per window position).
+constexpr int kOffHdr = 0, kOffLut = 64, kOffLev = kOffLut + 256, kOffSt = kOffLev + 256,
+              kOffFv = kOffSt + 264 * 2, kOffAcc = kOffFv + kRowOf * 4,
+              kOffTmp = kOffAcc + 64 * 4, kOffBig = kOffTmp + 64 * 4;
+static_assert(kOffBig % 16 == 0, "the big region is cleared and read in 16-byte words");
+
 struct FrArena {
   int32_t bytes;      // arena size (multiple of 16)
-  int32_t off_kb;     // uint32[p_max]   sort keys / zone keys
-  int32_t off_lvl;    // uint8[w_max]    compact level + 1 per window position
-  int32_t off_lut;    // uint8[256]      level -> compact index
-  int32_t off_lev;    // uint8[256]      compact index -> level
-  int32_t off_st;     // uint16[264]     start of each level run in the sorted keys
-  int32_t off_fv;     // float[96]       features of the current voxel
-  int32_t off_acc;    // float[32] + int32[32]  per-direction accumulators
-  int32_t off_tmp;    // float[64]       compensation terms of the direction sums
-  int32_t off_big;    // family matrices (layout from (mc, bc, w))
+  int32_t off_kb;     // uint32[p_max]
+  int32_t off_lvl;    // uint8[w_max]
   int32_t big_bytes;  // size of the shared big region
   int32_t p_max, w_max;
 };
@@ -189,13 +195,13 @@ struct BigLayout {
   int32_t bytes;
 };
 
-__host__ __device__ inline int32_t fr_align(int32_t v, int32_t a) {
+__host__ __device__ constexpr int32_t fr_align(int32_t v, int32_t a) {
   return (v + a - 1) / a * a;
 }
 
-__host__ __device__ inline BigLayout fr_big_layout(int32_t mc, int32_t bc,
+__host__ __device__ constexpr BigLayout fr_big_layout(int32_t mc, int32_t bc,
                                                    int32_t w) {
-  BigLayout L;
+  BigLayout L{};
   // GLCM
   L.cnt = 0;
   L.marg = L.cnt + mc * mc * 4;
@@ -247,27 +253,11 @@ inline FrArena fr_make_arena(int32_t r_max) {
   const int32_t s = 2 * r_max + 1;
   a.w_max = s * s * s;
   a.p_max = fr_next_pow2(a.w_max);
-  int32_t o = 0;
-  a.off_kb = o;
-  o += a.p_max * 4;
-  a.off_lvl = o;
-  o += fr_align(a.w_max, 16);
-  a.off_lut = o;
-  o += 256;
-  a.off_lev = o;
-  o += 256;
-  a.off_st = o;
-  o += 264 * 2;
-  a.off_fv = o;
-  o += kRowOf * 4;
-  a.off_acc = o;
-  o += 64 * 4;
-  a.off_tmp = o;
-  o += 64 * 4;
-  a.off_big = fr_align(o, 16);
   BigLayout L = fr_big_layout(kMCap, kBinCap, a.w_max);
   a.big_bytes = L.bytes;
-  a.bytes = fr_align(a.off_big + a.big_bytes, 16);
+  a.off_kb = fr_align(kOffBig + a.big_bytes, 16);
+  a.off_lvl = a.off_kb + a.p_max * 4;
+  a.bytes = fr_align(a.off_lvl + a.w_max, 16);
   return a;
 }
 

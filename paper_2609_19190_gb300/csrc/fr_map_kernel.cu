@@ -110,124 +110,112 @@ __device__ __noinline__ void feed(const FrMapArgs& args, Feeder& fd, int stage,
 }
 
 // Voxel t of the item, or no voxel (has == false: the warp only keeps step).
-// refill: this is the item's last round, so once every warp has gathered its
-// window the feeder reloads buffer `stage` (next barrier phase `parity`).
+// off: the warp's arena.  refill: this is the item's last round, so once every
+// warp has gathered its window the feeder reloads buffer `stage` (next barrier
+// phase `parity`).
 template <bool DUMP>
 __device__ __forceinline__ void map_voxel(const FrMapArgs& args, const FrJob& job,
-                                          const FrItem& item, const uint32_t* tile, int t, bool has,
-                                          Arena& A, char* smem_big, char* slab_big, int it, int nt,
-                                          Feeder& fd, bool refill, int stage, unsigned parity,
-                                          const FbPool& pool, unsigned char* arenas) {
+                                          const FrItem& item, int tile_off, int t, bool has,
+                                          int off, int it, int nt, Feeder& fd, bool refill,
+                                          int stage, unsigned parity, int pool_off,
+                                          int arenas_off) {
   const int lane = lane_id();
-  Win w;
   int col = 0;
   bool skip = false;
   int32_t *d_hist = nullptr, *d_glcm = nullptr, *d_glrlm = nullptr,
           *d_glszm = nullptr, *d_gldm = nullptr, *d_ngn = nullptr;
   long long* d_ngs = nullptr;
   if (has) {
+    VoxHdr* h = (VoxHdr*)(fr_smem + off);
     col = job.bcols[item.j0 + t];
     const int lin = job.voi[col];
     const int x = lin % job.nx;
     const int y = (lin / job.nx) % job.ny;
     const int z = lin / (job.nx * job.ny);
-    w.r = job.r;
-    w.s = 2 * job.r + 1;
-    w.s2 = w.s * w.s;
-    w.W = w.s2 * w.s;
-    w.ms.init((unsigned)w.s);
-    w.ms2.init((unsigned)w.s2);
-    w.ng = job.state->ng;
-    const int cx = (x - job.r) - (item.bx - job.hx);
-    const int cy = y - item.by;
-    const int cz = z - item.bz;
-    w.nv = gather_window(w, A, tile, job.box_x, job.box_y, cx, cy, cz);
-    // the big region is free until the families: the counting sort's bins
-    const bool counting = w.nv > kCsortMinKeys && w.nv <= 32 * kRadixRounds;
-    if (!counting || !warp_csort(A.kb, w.nv, (uint32_t*)smem_big, args.arena.big_bytes >> 2))
-      warp_sort_x(A.kb, w.nv, (int*)(A.tmp + 32));
+    if (lane == 0) {
+      h->r = job.r;
+      h->slab = nullptr;
+    }
+    __syncwarp();
+    int32_t* rec = nullptr;
     if (DUMP) {
-      const int ng = w.ng;
-      int32_t* rec = args.dbg + (size_t)it * args.dbg_stride;
+      const int ng = job.state->ng, s = 2 * job.r + 1, W = s * s * s;
+      rec = args.dbg + (size_t)it * args.dbg_stride;
       d_hist = rec + 4;
       d_glcm = d_hist + ng;
       d_glrlm = d_glcm + (size_t)kNumDirs * ng * ng;
-      d_glszm = d_glrlm + (size_t)kNumDirs * ng * w.s;
-      d_gldm = d_glszm + (size_t)ng * w.W;
+      d_glszm = d_glrlm + (size_t)kNumDirs * ng * s;
+      d_gldm = d_glszm + (size_t)ng * W;
       d_ngn = d_gldm + (size_t)ng * 27;
       size_t o = (size_t)(d_ngn + ng - rec);
       o = (o + 1) & ~(size_t)1;
       d_ngs = (long long*)(rec + o);
       if (lane == 0) {
         rec[0] = ng;
-        rec[1] = w.s;
-        rec[2] = w.W;
-        rec[3] = w.nv;
+        rec[1] = s;
+        rec[2] = W;
       }
     }
-    first_order(w, A, job, d_hist);
-    compact_levels(w, A);
-    if (w.m > kMCap || w.R >= kBinCap) {
-      if (slab_big == nullptr) {
+    vox_front<DUMP>(off, job, tile_off, (x - job.r) - (item.bx - job.hx), y - item.by, z - item.bz,
+                    d_hist, rec + 3);
+    if (h->m > kMCap || h->R >= kBinCap) {
+      char* slab = args.slab ? args.slab + ((size_t)blockIdx.x * args.consumer_warps +
+                                            (threadIdx.x >> 5)) * args.slab_stride
+                             : nullptr;
+      if (slab == nullptr) {
         if (lane == 0) atomicCAS(args.status, 0, kStatusUnsupported);
-        for (int f = lane; f < kNumFeatures; f += 32) A.fv[f] = kNaNf;
-        __syncwarp();
+        float* fv = (float*)(fr_smem + off + kOffFv);
+        for (int f = lane; f < kNumFeatures; f += 32) fv[f] = kNaNf;
         skip = true;
-      } else {
-        A.big = slab_big;
-        A.mc = args.slab_ngc;
-        A.bc = args.slab_ngc;
+      } else if (lane == 0) {
+        h->slab = slab;
+        h->ngc = args.slab_ngc;
       }
-    } else {
-      A.big = smem_big;
-      A.mc = kMCap;
-      A.bc = kBinCap;
+      __syncwarp();
     }
-    if (!skip) A.L = fr_big_layout(A.mc, A.bc, w.W);
   }
   const bool work = has && !skip;
   consumer_bar(nt);
   if (refill && threadIdx.x == 0) feed(args, fd, stage, parity);
   if (job.families & kFamGLCM) {
     const bool use_pool = args.fb != nullptr && (job.families & kFamMCC) != 0;
-    if (work) glcm_family(w, A, job, d_glcm, use_pool ? &pool : nullptr);
+    const float* fb = args.fb + (size_t)blockIdx.x * args.consumer_warps * args.fb_stride;
+    if (work)
+      vox_glcm<DUMP>(off, job, d_glcm, pool_off,
+                     use_pool ? (float*)fb + (threadIdx.x >> 5) * args.fb_stride : nullptr);
     if (use_pool) {
       consumer_bar(nt);  // the task list is complete
-      if (*(volatile int*)pool.count + *(volatile int*)pool.count_big > 0) {
-        const int s = 2 * job.r + 1;
-        fb_pool_work(pool, args, s * s * s, arenas, args.arena.bytes, args.arena.off_big, smem_big);
+      volatile int* pc = (volatile int*)(fr_smem + pool_off);
+      if (pc[0] + pc[2] > 0) {
+        fb_pool_work(pool_off, fb, args.fb_stride, arenas_off, args.arena.bytes);
         consumer_bar(nt);  // every radius is in its owner's results
-        if (threadIdx.x == 0) {
-          *pool.count = 0;
-          *pool.next = 0;
-          *pool.count_big = 0;
-          *pool.next_big = 0;
-        }
+        if (threadIdx.x == 0) pc[0] = pc[1] = pc[2] = pc[3] = 0;
       }
     }
-    if (work) glcm_finish(A, job);
+    if (work) vox_glcm_finish(off, job);
     consumer_bar(nt);
   }
   // GLRLM and GLSZM run without a barrier between them and GLDM: warps that
   // finish early go on (measured: the barriers after these two cost 1.5 %;
   // the ones after GLCM and GLDM keep the warps in the same code)
   if (job.families & kFamGLRLM) {
-    if (work) glrlm_family(w, A, job.agg == 1, d_glrlm);
+    if (work) vox_glrlm<DUMP>(off, job, d_glrlm);
   }
   if (job.families & kFamGLSZM) {
-    if (work) glszm_family(w, A, d_glszm);
+    if (work) vox_glszm<DUMP>(off, d_glszm);
   }
   if (job.families & (kFamGLDM | kFamNGTDM)) {
-    if (work) gldm_ngtdm_family(w, A, job, d_gldm, d_ngn, d_ngs);
+    if (work) vox_gldm<DUMP>(off, job, d_gldm, d_ngn, d_ngs);
     consumer_bar(nt);
   }
   if (has) {
     float* out = (float*)args.run_ptrs[2 * item.job + 1];
+    const float* fv = (const float*)(fr_smem + off + kOffFv);
     for (int f = lane; f < kNumFeatures; f += 32) {
       const int row = job.row_of[f];
       // maps are written once and never read here: streaming stores keep
       // them from evicting the MCC scratch from L2
-      if (row >= 0) __stcs(&out[(size_t)row * job.n_voi + col], A.fv[f]);
+      if (row >= 0) __stcs(&out[(size_t)row * job.n_voi + col], fv[f]);
     }
     __syncwarp();
   }
@@ -236,7 +224,7 @@ __device__ __forceinline__ void map_voxel(const FrMapArgs& args, const FrJob& jo
 template <bool DUMP>
 __global__ void __launch_bounds__(32 * kMaxConsumerWarps, 1)
     fr_map_kernel(const __grid_constant__ FrMapArgs args) {
-  extern __shared__ __align__(1024) unsigned char smem[];
+  unsigned char* const smem = fr_smem;
   const int S = args.stages, NW = args.consumer_warps;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const CtaLayout cl = fr_cta_layout(S, args.tile_bytes, NW, args.arena.bytes);
@@ -267,30 +255,15 @@ __global__ void __launch_bounds__(32 * kMaxConsumerWarps, 1)
   if (threadIdx.x == 0)
     for (int s = 0; s < S; ++s) feed(args, fd, s, 0u);
 
-  unsigned char* ab = smem + cl.arenas + warp * args.arena.bytes;
-  Arena A;
-  A.kb = (uint32_t*)(ab + args.arena.off_kb);
-  A.lvl = ab + args.arena.off_lvl;
-  A.lut = ab + args.arena.off_lut;
-  A.lev = ab + args.arena.off_lev;
-  A.st = (uint16_t*)(ab + args.arena.off_st);
-  A.fv = (float*)(ab + args.arena.off_fv);
-  A.facc = (float*)(ab + args.arena.off_acc);
-  A.nacc = (int*)(ab + args.arena.off_acc + 32 * 4);
-  A.tmp = (float*)(ab + args.arena.off_tmp);
-  A.fcomp = A.tmp;
-  char* smem_big = (char*)(ab + args.arena.off_big);
-  char* slab_big = args.slab ? args.slab + ((size_t)blockIdx.x * NW + warp) * args.slab_stride
-                             : nullptr;
+  const int off = cl.arenas + warp * args.arena.bytes;
+  if (lane == 0) {
+    VoxHdr* h = (VoxHdr*)(smem + off);
+    h->off_kb = args.arena.off_kb;
+    h->off_lvl = args.arena.off_lvl;
+    h->big_words = args.arena.big_bytes >> 2;
+  }
+  __syncwarp();
   const int nt = 32 * NW;
-  FbPool pool;
-  pool.count = (int*)(smem + cl.fb);
-  pool.next = pool.count + 1;
-  pool.count_big = pool.count + 2;
-  pool.next_big = pool.count + 3;
-  pool.tasks = pool.count + 4;
-  pool.scratch = args.fb ? args.fb + ((size_t)blockIdx.x * NW + warp) * args.fb_stride : nullptr;
-  pool.warp = warp;
   int stage = 0;
   unsigned phase = 0;
   while (true) {
@@ -312,12 +285,12 @@ __global__ void __launch_bounds__(32 * kMaxConsumerWarps, 1)
     if (it < 0) break;  // later buffers hold sentinels too: no copy in flight
     const FrItem item = args.items[it];
     const FrJob& job = args.jobs[item.job];
-    const uint32_t* tile = (const uint32_t*)(smem + cl.tiles + (size_t)stage * args.tile_bytes);
+    const int tile_off = cl.tiles + stage * args.tile_bytes;
     const int rounds = (item.n + NW - 1) / NW;
     for (int r = 0; r < rounds; ++r) {
       const int t = r * NW + warp;
-      map_voxel<DUMP>(args, job, item, tile, t, t < item.n, A, smem_big, slab_big, it, nt, fd,
-                      r == rounds - 1, stage, phase ^ 1u, pool, smem + cl.arenas);
+      map_voxel<DUMP>(args, job, item, tile_off, t, t < item.n, off, it, nt, fd,
+                      r == rounds - 1, stage, phase ^ 1u, cl.fb, cl.arenas);
     }
     if (++stage == S) {
       stage = 0;
