@@ -39,11 +39,13 @@ constexpr int kMaxConsumerWarps = 16;
 // bytes a row, with a zero row on every side.
 constexpr int kPadBytes = (7 + 2) * (7 + 2) * 8;
 constexpr int kMaxStages = 4;
-// CTA pool of many-level MCC solves: at most one per direction per warp;
-// each direction's S - u u^T is the packed upper triangle of its m x m
-// matrix (m (m + 1) / 2 contiguous floats, each written once) in the warp's
-// global scratch (kFbDir floats per direction)
+// CTA pool of MCC solves: at most one per direction per warp; with more than
+// kCapL levels a direction's S - u u^T is the packed upper triangle of its m x
+// m matrix (m (m + 1) / 2 contiguous floats, each written once) in the warp's
+// global scratch (kFbDir floats per direction).  kFbWords: 32-bit words of the
+// pool's counters (12) and lists.
 constexpr int kFbTasks = kMaxConsumerWarps * kNumDirs;
+constexpr int kFbWords = 12 + kFbTasks + 3 * kFbTasks / 2;
 constexpr int kFbDir = kMCap * kMCap;
 
 // Feature families (bits of FrJob::families).
@@ -115,6 +117,9 @@ struct FrItem {
 constexpr int kOffHdr = 0, kOffLut = 64, kOffLev = kOffLut + 256, kOffSt = kOffLev + 256,
               kOffFv = kOffSt + 264 * 2, kOffAcc = kOffFv + kRowOf * 4,
               kOffTmp = kOffAcc + 64 * 4, kOffBig = kOffTmp + 64 * 4;
+// MCC bookkeeping (rows, results; 16 words each) in tmp's second half, which
+// only the window sort uses
+constexpr int kOffMn = kOffTmp + 32 * 4;
 static_assert(kOffBig % 16 == 0, "the big region is cleared and read in 16-byte words");
 
 struct FrArena {
@@ -185,7 +190,7 @@ struct FrScalarArgs {
 // Big-region layout for caps (mc, bc) and window size w.
 struct BigLayout {
   int32_t cnt, marg, prank, sbin, dbin, vec;  // GLCM (vec: 4 float vectors of mc)
-  int32_t mn, mres, slots;                    // GLCM MCC: n per direction, results, slots
+  int32_t slots;                              // GLCM MCC: the directions' matrices
   int32_t csn, cst;                           // GLCM ClusterShade numerators (f64), totals
   int32_t rhist, rlv, rlen;                  // GLRLM
   int32_t parent, zsz, zlv;                  // GLSZM
@@ -208,9 +213,7 @@ __host__ __device__ constexpr BigLayout fr_big_layout(int32_t mc, int32_t bc,
   L.sbin = L.prank + mc * 4;
   L.dbin = L.sbin + 2 * bc * 4;
   L.vec = L.dbin + bc * 4;
-  L.mn = L.vec + 4 * mc * 4;
-  L.mres = L.mn + 16 * 4;
-  L.slots = L.mres + 16 * 4;
+  L.slots = fr_align(L.vec + 4 * mc * 4, 16);
   L.csn = fr_align(L.slots + kNumDirs * kSlot * 4, 8);
   L.cst = L.csn + 16 * 8;
   int32_t glcm_end = L.cst + 16 * 4;

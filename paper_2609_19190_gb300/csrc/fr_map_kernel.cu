@@ -32,8 +32,8 @@ __host__ __device__ inline CtaLayout fr_cta_layout(int stages, int tile_bytes,
   c.tiles = 0;
   c.bars = stages * tile_bytes;
   c.slots = c.bars + 2 * stages * 8;
-  c.fb = c.slots + stages * 4;  // pool: count, next, count_big, next_big, kFbTasks tasks
-  c.arenas = fr_align(c.fb + (4 + kFbTasks) * 4, 128);
+  c.fb = c.slots + stages * 4;  // pool: counters and lists
+  c.arenas = fr_align(c.fb + kFbWords * 4, 128);
   c.bytes = c.arenas + nw * arena_bytes;
   return c;
 }
@@ -183,13 +183,14 @@ __device__ __forceinline__ void map_voxel(const FrMapArgs& args, const FrJob& jo
     if (work)
       vox_glcm<DUMP>(off, job, d_glcm, pool_off,
                      use_pool ? (float*)fb + (threadIdx.x >> 5) * args.fb_stride : nullptr);
+    if (work && use_pool) pool_list_slots(pool_off, off);
     if (use_pool) {
       consumer_bar(nt);  // the task list is complete
-      volatile int* pc = (volatile int*)(fr_smem + pool_off);
-      if (pc[0] + pc[2] > 0) {
+      const volatile int* pc = (const volatile int*)(fr_smem + pool_off);
+      if (pc[0] + pc[1] + pc[2] + pc[3] + pc[4] > 0) {
         fb_pool_work(pool_off, fb, args.fb_stride, arenas_off, args.arena.bytes);
         consumer_bar(nt);  // every radius is in its owner's results
-        if (threadIdx.x == 0) pc[0] = pc[1] = pc[2] = pc[3] = 0;
+        if (threadIdx.x < 10) ((volatile int*)pc)[threadIdx.x] = 0;
       }
     }
     if (work) vox_glcm_finish(off, job);
@@ -244,7 +245,7 @@ __global__ void __launch_bounds__(32 * kMaxConsumerWarps, 1)
     for (int s = 0; s < S; ++s) mbar_init(&fd.full[s], 1);
     fence_mbar_init();
     int* fbc = (int*)(smem + cl.fb);
-    for (int q = 0; q < 4; ++q) fbc[q] = 0;
+    for (int q = 0; q < 10; ++q) fbc[q] = 0;
   }
   // zero this warp's arena (the count matrices must start at zero)
   {
