@@ -109,6 +109,15 @@ __device__ __noinline__ void feed(const FrMapArgs& args, Feeder& fd, int stage,
   fd.ppar[stage] = parity;
 }
 
+// What a warp carries from one voxel to the next: the voxel it maps next, if
+// known (item it, index t in the item, column, linear voxel index), and its
+// lanes' output rows in the last job.
+struct NextVoxel {
+  int it, t, col, lin;
+  int job;
+  int row[4];
+};
+
 // Voxel t of the item, or no voxel (has == false: the warp only keeps step).
 // off: the warp's arena.  refill: this is the item's last round, so once every
 // warp has gathered its window the feeder reloads buffer `stage` (next barrier
@@ -116,7 +125,8 @@ __device__ __noinline__ void feed(const FrMapArgs& args, Feeder& fd, int stage,
 template <bool DUMP>
 __device__ __forceinline__ void map_voxel(const FrMapArgs& args, const FrJob& job,
                                           const FrItem& item, int tile_off, int t, bool has,
-                                          int off, int it, int nt, Feeder& fd, bool refill,
+                                          int off, int it, int nt, Feeder& fd, NextVoxel& nx,
+                                          bool refill,
                                           int stage, unsigned parity, int pool_off,
                                           int arenas_off) {
   const int lane = lane_id();
@@ -127,8 +137,9 @@ __device__ __forceinline__ void map_voxel(const FrMapArgs& args, const FrJob& jo
   long long* d_ngs = nullptr;
   if (has) {
     VoxHdr* h = (VoxHdr*)(fr_smem + off);
-    col = job.bcols[item.j0 + t];
-    const int lin = job.voi[col];
+    const bool ahead = nx.it == it && nx.t == t;
+    col = ahead ? nx.col : job.bcols[item.j0 + t];
+    const int lin = ahead ? nx.lin : job.voi[col];
     const int x = lin % job.nx;
     const int y = (lin / job.nx) % job.ny;
     const int z = lin / (job.nx * job.ny);
@@ -209,15 +220,38 @@ __device__ __forceinline__ void map_voxel(const FrMapArgs& args, const FrJob& jo
     if (work) vox_gldm<DUMP>(off, job, d_gldm, d_ngn, d_ngs);
     consumer_bar(nt);
   }
+  // this warp's next voxel: its column and position are two dependent reads
+  // away, which the stores below hide (4k cycles of a voxel's 120k at r = 1).
+  // The next item is known where a barrier lies between the feeder's claim
+  // and here.
+  if (refill && (job.families & (kFamGLCM | kFamGLDM | kFamNGTDM))) {
+    const int it2 = fd.slot[stage + 1 == args.stages ? 0 : stage + 1], t2 = (int)threadIdx.x >> 5;
+    nx.it = -1;
+    if (it2 >= 0 && it2 < args.n_items) {
+      const FrItem& i2 = args.items[it2];
+      if (t2 < i2.n) {
+        const FrJob& j2 = args.jobs[i2.job];
+        nx.col = j2.bcols[i2.j0 + t2];
+        nx.lin = j2.voi[nx.col];
+        nx.it = it2;
+        nx.t = t2;
+      }
+    }
+  }
   if (has) {
-    float* out = (float*)args.run_ptrs[2 * item.job + 1];
+    if (nx.job != item.job) {  // the output rows of this lane's features
+      nx.job = item.job;
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        nx.row[k] = 32 * k + lane < kNumFeatures ? job.row_of[32 * k + lane] : -1;
+    }
+    float* out = (float*)args.run_ptrs[2 * item.job + 1] + col;
     const float* fv = (const float*)(fr_smem + off + kOffFv);
-    for (int f = lane; f < kNumFeatures; f += 32) {
-      const int row = job.row_of[f];
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
       // maps are written once and never read here: streaming stores keep
       // them from evicting the MCC scratch from L2
-      if (row >= 0) __stcs(&out[(size_t)row * job.n_voi + col], fv[f]);
-    }
+      if (nx.row[k] >= 0) __stcs(&out[(size_t)nx.row[k] * job.n_voi], fv[32 * k + lane]);
     __syncwarp();
   }
 }
@@ -265,6 +299,8 @@ __global__ void __launch_bounds__(32 * kMaxConsumerWarps, 1)
   }
   __syncwarp();
   const int nt = 32 * NW;
+  NextVoxel nx;
+  nx.it = nx.t = nx.col = nx.lin = nx.job = -1;
   int stage = 0;
   unsigned phase = 0;
   while (true) {
@@ -290,7 +326,7 @@ __global__ void __launch_bounds__(32 * kMaxConsumerWarps, 1)
     const int rounds = (item.n + NW - 1) / NW;
     for (int r = 0; r < rounds; ++r) {
       const int t = r * NW + warp;
-      map_voxel<DUMP>(args, job, item, tile_off, t, t < item.n, off, it, nt, fd,
+      map_voxel<DUMP>(args, job, item, tile_off, t, t < item.n, off, it, nt, fd, nx,
                       r == rounds - 1, stage, phase ^ 1u, cl.fb, cl.arenas);
     }
     if (++stage == S) {
