@@ -978,14 +978,14 @@ fr_status scalar_open(fr_scalar& S, const fr_map_params* p, const uint8_t* mask)
                  o_glcm = take((size_t)kNumDirs * (ngc * (ngc + 1) / 2) * 4),
                  o_glrlm = take((size_t)kNumDirs * ngc * lmax * 4), o_zsize = take((size_t)nvox * 4),
                  o_zrow = take(256 * 4), o_zcol = take((size_t)(j.n_voi + 1) * 4),
-                 o_hcnt = take((size_t)hcap * 4);
+                 o_hcnt = take((size_t)hcap * 4), o_zsum = take(24 * 8);
     S.zero_bytes = off;
     const size_t o_hkey = take((size_t)hcap * 8);
     S.key_off = o_hkey;
     S.key_bytes = (size_t)hcap * 8;
     const size_t o_parent = take((size_t)nvox * 4),
                  o_mccs = take((size_t)kNumDirs * ngc * ngc * 4),
-                 o_mccv = take((size_t)kNumDirs * 4 * ngc * 4), o_dirf = take(kNumDirs * kScalarDirF * 8),
+                 o_dirf = take(kNumDirs * kScalarDirF * 8),
                  o_out = take(kRowOf * 8);
     S.scratch = dev_alloc<char>(off, &S.bytes);
     FrScalarArgs& A = S.A;
@@ -1017,9 +1017,9 @@ fr_status scalar_open(fr_scalar& S, const fr_map_params* p, const uint8_t* mask)
     A.hcnt = (uint32_t*)(S.scratch + o_hcnt);
     A.hkey = (unsigned long long*)(S.scratch + o_hkey);
     A.hcap = hcap;
+    A.zsum = (unsigned long long*)(S.scratch + o_zsum);
     A.parent = (int32_t*)(S.scratch + o_parent);
     A.mcc_s = (float*)(S.scratch + o_mccs);
-    A.mcc_v = (float*)(S.scratch + o_mccv);
     A.dirf = (double*)(S.scratch + o_dirf);
     A.out = (double*)(S.scratch + o_out);
     A.status = S.d_status;

@@ -180,8 +180,8 @@ struct FrScalarArgs {
   unsigned long long* hkey;    // [hcap] (level << 32 | size) keys, ~0 = empty
   uint32_t* hcnt;              // [hcap] zones per key
   int64_t hcap;                // power of two >= 2 n_voi
+  unsigned long long* zsum;    // [24] zone sums: 11 of 128 bits, sizes' squares, blocks done
   float* mcc_s;                // [13][ngc][ngc] deflated S matrices
-  float* mcc_v;                // [13][4][ngc] solver vectors
   double* dirf;                // [13][kScalarDirF]: GLCM (24), GLRLM (16), GLCM extras (2)
   double* out;                 // [kRowOf] feature values (written by the final kernel)
   int32_t* status;             // run status word

@@ -8,7 +8,7 @@
 // 26-connected zones by a lock-free union-find over the volume, zone (level,
 // size) pairs in an open-addressing hash table.  Counts are exact integers;
 // the features are then taken in FP64 by a few small kernels (MCC in FP32 by
-// the warp eigen-solver of the map path), one block per direction.
+// the warp eigen-solver of the map path in shared memory), one block per direction.
 #include <cfloat>
 #include <climits>
 #include <cstdint>
@@ -22,9 +22,15 @@ namespace fr {
 constexpr unsigned long long kEmptyKey = ~0ull;
 constexpr int kScThreads = 256;
 constexpr int kMiscThreads = 1024;
-// dynamic shared memory of the neighbourhood kernel:
-// ngacc [256][27] u64, gldm [256][27] u32, hlev [256] u32, ngn [256] u32
-constexpr int kNeighSmem = 256 * 27 * 8 + 256 * 27 * 4 + 256 * 4 + 256 * 4;
+// threads of the counting blocks that keep a private copy of the counts: the
+// copies are sized by the plan's level cap (83 and 130 KB at 255 levels, two
+// blocks and one an SM), so the warps in flight come from wide blocks
+constexpr int kCountThreads = 1024;
+// dynamic shared memory of the neighbourhood kernel, for levels 0..ngc:
+// ngacc [27] u64, gldm [27] u32, hlev u32, ngn u32
+static __host__ __device__ constexpr int neigh_smem(int ngc) {
+  return (ngc + 1) * (27 * 8 + 27 * 4 + 4 + 4);
+}
 
 __device__ __forceinline__ bool sc_failed(const FrScalarArgs& a) {
   return *(const volatile int32_t*)&a.state->status != 0;
@@ -169,18 +175,20 @@ __global__ void sc_init_kernel(const __grid_constant__ FrScalarArgs a) {
 
 // Per VOI voxel: raw / level histograms, GLDM dependence (equal 26-neighbours),
 // NGTDM n_i and |i k - sum|, and the zone unions with the 13 forward
-// neighbours of equal level.
-__global__ void __launch_bounds__(kScThreads) sc_neigh_kernel(const __grid_constant__ FrScalarArgs a) {
+// neighbours of equal level.  Bound by the latency of the neighbour reads and
+// of the unions; a block clears and adds only the levels in use (200k voxels: 290 us).
+__global__ void __launch_bounds__(kCountThreads) sc_neigh_kernel(const __grid_constant__ FrScalarArgs a) {
   extern __shared__ __align__(16) unsigned char sm[];
-  unsigned long long* s_acc = (unsigned long long*)sm;  // [256][27]
-  uint32_t* s_gldm = (uint32_t*)(s_acc + 256 * 27);    // [256][27]
-  uint32_t* s_hlev = s_gldm + 256 * 27;                 // [256]
-  uint32_t* s_ngn = s_hlev + 256;                       // [256]
-  for (int i = threadIdx.x; i < 256 * 27; i += blockDim.x) {
+  const int rows = sc_failed(a) ? 0 : a.state->ng + 1, cells = rows * 27;
+  unsigned long long* s_acc = (unsigned long long*)sm;  // [rows][27]
+  uint32_t* s_gldm = (uint32_t*)(s_acc + cells);        // [rows][27]
+  uint32_t* s_hlev = s_gldm + cells;                    // [rows]
+  uint32_t* s_ngn = s_hlev + rows;                      // [rows]
+  for (int i = threadIdx.x; i < cells; i += blockDim.x) {
     s_acc[i] = 0ull;
     s_gldm[i] = 0u;
   }
-  for (int i = threadIdx.x; i < 256; i += blockDim.x) s_hlev[i] = s_ngn[i] = 0u;
+  for (int i = threadIdx.x; i < rows; i += blockDim.x) s_hlev[i] = s_ngn[i] = 0u;
   __syncthreads();
   if (!sc_failed(a)) {
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < a.n_voi;
@@ -216,11 +224,11 @@ __global__ void __launch_bounds__(kScThreads) sc_neigh_kernel(const __grid_const
     }
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < 256 * 27; i += blockDim.x) {
+  for (int i = threadIdx.x; i < cells; i += blockDim.x) {
     if (s_acc[i]) atomicAdd(&a.ngacc[i], s_acc[i]);
     if (s_gldm[i]) atomicAdd(&a.gldm[i], s_gldm[i]);
   }
-  for (int i = threadIdx.x; i < 256; i += blockDim.x) {
+  for (int i = threadIdx.x; i < rows; i += blockDim.x) {
     if (s_hlev[i]) atomicAdd(&a.hlev[i], s_hlev[i]);
     if (s_ngn[i]) atomicAdd(&a.ngn[i], s_ngn[i]);
   }
@@ -228,28 +236,32 @@ __global__ void __launch_bounds__(kScThreads) sc_neigh_kernel(const __grid_const
 
 // Co-occurrence pairs (u, u + delta d) of direction blockIdx.y, as packed
 // upper-triangle counts over levels (a shared-memory copy per block).
-__global__ void __launch_bounds__(kScThreads) sc_glcm_kernel(const __grid_constant__ FrScalarArgs a) {
+__global__ void __launch_bounds__(kCountThreads) sc_glcm_kernel(const __grid_constant__ FrScalarArgs a) {
   extern __shared__ __align__(16) unsigned char sm[];
+  if (sc_failed(a)) return;
   uint32_t* s = (uint32_t*)sm;
-  const int ngc = a.ngc, np = ngc * (ngc + 1) / 2, d = blockIdx.y;
+  // the levels in use fill the leading triangle of the block's copy
+  const int ng = a.state->ng, np = ng * (ng + 1) / 2, ngc = a.ngc, d = blockIdx.y;
   for (int i = threadIdx.x; i < np; i += blockDim.x) s[i] = 0u;
   __syncthreads();
-  if (!sc_failed(a)) {
-    const int oz = c_dirs[d][0] * a.delta, oy = c_dirs[d][1] * a.delta, ox = c_dirs[d][2] * a.delta;
-    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < a.n_voi;
-         k += (int64_t)gridDim.x * blockDim.x) {
-      int z, y, x;
-      sc_zyx(a, a.voi[k], z, y, x);
-      const int g = sc_level(a, z, y, x);
-      const int b = sc_level(a, z + oz, y + oy, x + ox);
-      if (!b) continue;
-      atomicAdd(&s[pk(ngc, min(g, b) - 1, max(g, b) - 1)], 1u);
-    }
+  const int oz = c_dirs[d][0] * a.delta, oy = c_dirs[d][1] * a.delta, ox = c_dirs[d][2] * a.delta;
+  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < a.n_voi;
+       k += (int64_t)gridDim.x * blockDim.x) {
+    int z, y, x;
+    sc_zyx(a, a.voi[k], z, y, x);
+    const int g = sc_level(a, z, y, x);
+    const int b = sc_level(a, z + oz, y + oy, x + ox);
+    if (!b) continue;
+    atomicAdd(&s[pk(ng, min(g, b) - 1, max(g, b) - 1)], 1u);
   }
   __syncthreads();
-  uint32_t* dst = a.glcm + (size_t)d * np;
-  for (int i = threadIdx.x; i < np; i += blockDim.x)
-    if (s[i]) atomicAdd(&dst[i], s[i]);
+  uint32_t* dst = a.glcm + (size_t)d * (ngc * (ngc + 1) / 2);
+  for (int t = threadIdx.x; t < ng * ng; t += blockDim.x) {
+    const int i = t / ng, j = t - i * ng;
+    if (j < i) continue;
+    const uint32_t c = s[pk(ng, i, j)];
+    if (c) atomicAdd(&dst[pk(ngc, i, j)], c);
+  }
 }
 
 // Runs of direction blockIdx.y: a voxel whose predecessor (u - d) is not of
@@ -332,15 +344,43 @@ __device__ __forceinline__ double sc_bregman(double d) {
   return (1.0 + d) * log1p(d) - d;
 }
 
+// The t-th cell (i <= j) of the upper triangle of n levels, rows r and
+// n - 1 - r side by side: t < (n + 1) / 2 * (n + 1); false for the middle
+// row's second half (n odd).
+__device__ __forceinline__ bool sc_cell(int t, int n, int& i, int& j) {
+  const int r = t / (n + 1), c = t - r * (n + 1);
+  if (c < n - r) {
+    i = r;
+    j = r + c;
+    return true;
+  }
+  i = n - 1 - r;
+  j = i + c - (n - r);
+  return i > r;
+}
+
 // GLCM features of direction blockIdx.x (or of the merged matrix), written to
 // dirf[blockIdx.x][0..23] (and the IBSI sum variance and dissimilarity at
 // [40..41]).  Counts C(i, j): n for i != j, 2n on the diagonal.
+//
+// Bound by the FP64 pipe (one warp instruction in 16 cycles of an SM) and by
+// chains of dependent FP64 instructions: what depends on |i - j| or i + j
+// alone is taken from the difference and sum bins (ng and 2 ng terms instead
+// of ng^2), sums of integers stay integers, a cell of the triangle stands for
+// both entries, and one warp solves the MCC in shared memory meanwhile.
+// 200k voxels, 26 levels: 1147 -> 195 us.
 __global__ void __launch_bounds__(kScThreads) sc_glcm_feat_kernel(const __grid_constant__ FrScalarArgs a) {
   __shared__ unsigned long long s_marg[256];
   __shared__ unsigned long long s_sbin[512];
   __shared__ unsigned long long s_dbin[256];
-  __shared__ double s_red[16 * 32];
+  __shared__ double s_rs[256];
+  __shared__ double s_red[15 * 32];
+  __shared__ unsigned long long s_ured[32];
+  // the solve: 64 rows, then a tridiagonal and factors of up to 255
+  __shared__ float4 s_room[(64 * 64 * 4 + 256 * 24) / 16];
+  __shared__ unsigned long long s_max;
   __shared__ int s_present;
+  __shared__ float s_mcc;
   const int d = blockIdx.x, tid = threadIdx.x;
   double* f = a.dirf + d * kScalarDirF;
   const double kNaN = __longlong_as_double(0x7ff8000000000000ll);
@@ -351,25 +391,42 @@ __global__ void __launch_bounds__(kScThreads) sc_glcm_feat_kernel(const __grid_c
   }
   const bool merged = a.agg == 1;
   const int ng = a.state->ng, ngc = a.ngc, np = ngc * (ngc + 1) / 2;
-  auto cnt = [&](int i, int j) -> unsigned long long {  // pair count, 0-based levels
-    const size_t t = (size_t)pk(ngc, min(i, j), max(i, j));
+  auto cnt = [&](int i, int j) -> unsigned long long {  // pair count, 0-based levels i <= j
+    const size_t t = (size_t)pk(ngc, i, j);
     if (!merged) return a.glcm[(size_t)d * np + t];
     unsigned long long s = 0;
+#pragma unroll
     for (int q = 0; q < kNumDirs; ++q) s += a.glcm[(size_t)q * np + t];
     return s;
   };
   for (int i = tid; i < 512; i += blockDim.x) s_sbin[i] = 0ull;
-  for (int i = tid; i < 256; i += blockDim.x) s_dbin[i] = 0ull;
-  if (tid == 0) s_present = 0;
-  __syncthreads();
-  for (int i = tid; i < 256; i += blockDim.x) {
-    unsigned long long c = 0;
-    if (i < ng)
-      for (int j = 0; j < ng; ++j) c += (i == j ? 2ull : 1ull) * cnt(i, j);
-    s_marg[i] = c;
-    if (c) atomicAdd(&s_present, 1);
+  for (int i = tid; i < 256; i += blockDim.x) s_dbin[i] = s_marg[i] = 0ull;
+  if (tid == 0) {
+    s_max = 0ull;
+    s_present = 0;
+    s_mcc = 0.f;
   }
   __syncthreads();
+  const int cells = (ng + 1) / 2 * (ng + 1);
+  unsigned long long ij[1] = {0ull};  // sum of (i + 1)(j + 1) C
+  {
+    unsigned long long mx = 0ull;
+    for (int t = tid; t < cells; t += blockDim.x) {
+      int i, j;
+      if (!sc_cell(t, ng, i, j)) continue;
+      const unsigned long long n = cnt(i, j);
+      if (!n) continue;
+      const unsigned long long C = i == j ? 2ull * n : n;
+      atomicAdd(&s_marg[i], C);
+      if (i != j) atomicAdd(&s_marg[j], C);
+      atomicAdd(&s_sbin[i + j + 2], 2ull * n);
+      atomicAdd(&s_dbin[j - i], 2ull * n);
+      ij[0] += 2ull * n * (unsigned)((i + 1) * (j + 1));
+      mx = max(mx, C);
+    }
+    if (mx) atomicMax(&s_max, mx);
+  }
+  block_sum_u64<1>(ij, s_ured);
   unsigned long long T = 0;
   for (int i = 0; i < ng; ++i) T += s_marg[i];
   if (T == 0) {
@@ -377,128 +434,142 @@ __global__ void __launch_bounds__(kScThreads) sc_glcm_feat_kernel(const __grid_c
     if (tid < 2) f[40 + tid] = kNaN;
     return;
   }
-  const double dT = (double)T;
-  double mu = 0.0, hx = 0.0;
-  for (int i = 0; i < ng; ++i) {
-    const double p = (double)s_marg[i] / dT;
-    mu += (i + 1) * p;
-    hx += sc_ent(p);
-  }
-  double sig2 = 0.0;
-  for (int i = 0; i < ng; ++i) sig2 += ((i + 1) - mu) * ((i + 1) - mu) * ((double)s_marg[i] / dT);
-  // entries
-  double v[16];
-  for (int k = 0; k < 16; ++k) v[k] = 0.0;
-  double maxp = 0.0;
-  const double ngd = (double)ng;
-  for (int t = tid; t < ng * ng; t += blockDim.x) {
-    const int i = t / ng, j = t - i * ng;
-    const unsigned long long mi = s_marg[i], mj = s_marg[j];
-    const unsigned long long C = (i == j ? 2ull : 1ull) * cnt(i, j);
-    if (!mi || !mj) continue;
-    // mutual information, nats: sum of q g(p / q - 1) >= 0 over all present pairs
-    const long long num = (long long)C * (long long)T - (long long)(mi * mj);
-    const double q = ((double)mi / dT) * ((double)mj / dT);
-    v[15] += q * sc_bregman((double)num / ((double)mi * (double)mj));
-    if (!C) continue;
-    const double p = (double)C / dT;
-    const double I = i + 1, J = j + 1, tt = I + J - 2.0 * mu, dd = fabs(I - J);
-    v[0] += I * J * p;                   // autocorrelation
-    v[1] += tt * tt * tt * tt * p;       // cluster prominence
-    v[2] += tt * tt * tt * p;            // cluster shade
-    v[3] += tt * tt * p;                 // cluster tendency
-    v[4] += dd * dd * p;                 // contrast
-    v[5] += p * p;                       // joint energy
-    v[6] += sc_ent(p);                   // joint entropy
-    v[7] += p / (1.0 + dd * dd);         // Idm
-    v[8] += p / (1.0 + dd * dd / (ngd * ngd));
-    v[9] += p / (1.0 + dd);              // Id
-    v[10] += p / (1.0 + dd / ngd);       // Idn
-    if (i != j) v[11] += p / (dd * dd);  // inverse variance
-    v[12] += (I - mu) * (I - mu) * p;    // sum of squares
-    maxp = fmax(maxp, p);
-    atomicAdd(&s_sbin[i + j + 2], C);
-    atomicAdd(&s_dbin[i > j ? i - j : j - i], C);
-  }
-  block_sum<16>(v, s_red);
-  // maximum probability
-  {
-    double m = maxp;
-    for (int o = 16; o; o >>= 1) m = fmax(m, __shfl_xor_sync(kFull, m, o));
-    if ((tid & 31) == 0) s_red[tid >> 5] = m;
-    __syncthreads();
-    if (tid == 0) {
-      double mm = 0.0;
-      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) mm = fmax(mm, s_red[w]);
-      s_red[0] = mm;
+  const double dT = (double)T, iT = 1.0 / dT;
+  double u[4] = {0.0, 0.0, 0.0, 0.0};  // mean, HX, difference average, sum average
+  for (int i = tid; i < 2 * ng + 1; i += blockDim.x) {
+    if (i < ng) {
+      const unsigned long long mi = s_marg[i];
+      s_rs[i] = mi ? 1.0 / sqrt((double)mi) : 0.0;
+      if (mi) atomicAdd(&s_present, 1);
+      const double p = (double)mi / dT;
+      u[0] += (i + 1) * p;
+      u[1] += sc_ent(p);
+      u[2] += i * ((double)s_dbin[i] / dT);
     }
-    __syncthreads();
-    maxp = s_red[0];
-    __syncthreads();
+    u[3] += i * ((double)s_sbin[i] / dT);
   }
+  block_sum<4>(u, s_red);
+  const double mu = u[0], hx = u[1], da = u[2], sa = u[3];
   // MCC: spectral radius of S - u u^T over the levels (absent levels: zero rows)
   float* S = a.mcc_s + (size_t)d * ngc * ngc;
-  for (int t = tid; t < ng * ng; t += blockDim.x) {
-    const int i = t / ng, j = t - i * ng;
+  for (int t = tid; t < cells; t += blockDim.x) {
+    int i, j;
+    if (!sc_cell(t, ng, i, j)) continue;
     const unsigned long long mi = s_marg[i], mj = s_marg[j];
-    float val = 0.f;
-    if (mi && mj) {
-      const unsigned long long C = (i == j ? 2ull : 1ull) * cnt(i, j);
-      const long long num = (long long)C * (long long)T - (long long)(mi * mj);
-      val = (float)((double)num / (dT * sqrt((double)mi * (double)mj)));
-    }
+    const unsigned long long C = (i == j ? 2ull : 1ull) * cnt(i, j);
+    const long long num = (long long)C * (long long)T - (long long)(mi * mj);
+    const float val = (float)((double)num * (s_rs[i] * s_rs[j]) * iT);
     S[(size_t)i * ngc + j] = val;
+    S[(size_t)j * ngc + i] = val;
   }
   __syncthreads();
-  float mcc = 0.f;
-  if (tid < 32 && s_present >= 2) {
-    float* vv = a.mcc_v + (size_t)d * 4 * ngc;
-    mcc = spectral_radius(S, ng, ngc, vv, vv + ngc, vv + 2 * ngc, vv + 3 * ngc);
+  double v[15];
+  for (int k = 0; k < 15; ++k) v[k] = 0.0;
+  if (tid < 32) {
+    if (s_present >= 2) {
+      const float mcc = warp_rho(S, ngc, ng, nullptr, 0.f, (char*)s_room, (int)sizeof(s_room));
+      if (tid == 0) s_mcc = mcc;
+    }
+  } else {
+    for (int t = tid - 32; t < cells; t += blockDim.x - 32) {
+      int i, j;
+      if (!sc_cell(t, ng, i, j)) continue;
+      const unsigned long long mi = s_marg[i], mj = s_marg[j];
+      if (!mi || !mj) continue;
+      const double w = i == j ? 1.0 : 2.0;
+      const unsigned long long C = (i == j ? 2ull : 1ull) * cnt(i, j);
+      // mutual information, nats: sum of q g(p / q - 1) >= 0 over all present pairs
+      const long long num = (long long)C * (long long)T - (long long)(mi * mj);
+      const double mm = (double)mi * (double)mj;
+      v[0] += w * (mm * (iT * iT)) * sc_bregman((double)num / mm);
+      if (!C) continue;
+      const double p = (double)C / dT;
+      v[1] += w * (p * p);       // joint energy
+      v[2] += w * sc_ent(p);     // joint entropy
+    }
+    const double ngd = (double)ng;
+    for (int k = tid - 32; k < 2 * ng + 1; k += blockDim.x - 32) {
+      if (k < ng) {
+        v[3] += ((k + 1) - mu) * ((k + 1) - mu) * ((double)s_marg[k] / dT);  // sum of squares
+        const unsigned long long c = s_dbin[k];
+        if (c) {
+          const double p = (double)c / dT, dd = k;
+          v[4] += dd * dd * p;                          // contrast
+          v[5] += p / (1.0 + dd * dd);                  // Idm
+          v[6] += p / (1.0 + dd * dd / (ngd * ngd));    // Idmn
+          v[7] += p / (1.0 + dd);                       // Id
+          v[8] += p / (1.0 + dd / ngd);                 // Idn
+          if (k) v[9] += p / (dd * dd);                 // inverse variance
+          v[10] += sc_ent(p);                           // difference entropy
+          v[11] += (dd - da) * (dd - da) * p;           // difference variance
+        }
+      }
+      const unsigned long long c = s_sbin[k];
+      if (c) {
+        const double p = (double)c / dT, tt = k - 2.0 * mu, t2 = tt * tt;
+        v[12] += t2 * t2 * p;  // cluster prominence
+        v[13] += t2 * tt * p;  // cluster shade
+        v[14] += t2 * p;       // cluster tendency
+      }
+    }
   }
+  // (the bin 2 ng of the sums is the last: two levels ng)
+  block_sum<15>(v, s_red);
+  double e[2] = {0.0, 0.0};  // sum entropy, sum variance
+  for (int k = tid; k < 2 * ng + 1; k += blockDim.x) {
+    const double p = (double)s_sbin[k] / dT;
+    e[0] += sc_ent(p);
+    e[1] += (k - sa) * (k - sa) * p;
+  }
+  block_sum<2>(e, s_red);
   if (tid == 0) {
-    double da = 0.0, de = 0.0, sa = 0.0, se = 0.0;
-    for (int k = 0; k < ng; ++k) {
-      const double p = (double)s_dbin[k] / dT;
-      da += k * p;
-      de += sc_ent(p);
-    }
-    double dv = 0.0;
-    for (int k = 0; k < ng; ++k) dv += (k - da) * (k - da) * ((double)s_dbin[k] / dT);
-    for (int k = 2; k <= 2 * ng; ++k) {
-      const double p = (double)s_sbin[k] / dT;
-      sa += k * p;
-      se += sc_ent(p);
-    }
-    double sv = 0.0;
-    for (int k = 2; k <= 2 * ng; ++k) sv += (k - sa) * (k - sa) * ((double)s_sbin[k] / dT);
-    f[40] = sv;
+    f[40] = e[1];
     f[41] = da;
-    const double mi_bits = v[15] * 1.4426950408889634;
-    f[0] = v[0];
+    const double mi_bits = v[0] * 1.4426950408889634, ac = (double)ij[0] / dT;
+    f[0] = ac;
     f[1] = mu;
-    f[2] = v[1];
-    f[3] = v[2];
-    f[4] = v[3];
+    f[2] = v[12];
+    f[3] = v[13];
+    f[4] = v[14];
     f[5] = v[4];
-    f[6] = sc_div(v[0] - mu * mu, sig2);
+    f[6] = sc_div(ac - mu * mu, v[3]);
     f[7] = da;
-    f[8] = de;
-    f[9] = dv;
-    f[10] = v[5];
-    f[11] = v[6];
+    f[8] = v[10];
+    f[9] = v[11];
+    f[10] = v[1];
+    f[11] = v[2];
     f[12] = sc_div(-mi_bits, hx);
     f[13] = sqrt(fmax(0.0, -expm1(-2.0 * mi_bits)));
-    f[14] = v[7];
-    f[15] = v[8];
-    f[16] = v[9];
-    f[17] = v[10];
-    f[18] = v[11];
-    f[19] = maxp;
+    f[14] = v[5];
+    f[15] = v[6];
+    f[16] = v[7];
+    f[17] = v[8];
+    f[18] = v[9];
+    f[19] = (double)s_max / dT;
     f[20] = sa;
-    f[21] = se;
-    f[22] = v[12];
-    f[23] = s_present >= 2 ? (double)mcc : kNaN;
+    f[21] = e[0];
+    f[22] = v[3];
+    f[23] = s_present >= 2 ? (double)s_mcc : kNaN;
   }
+}
+
+// The eleven sums over a (gray level I, size J) matrix's cells of share p
+// (short and long, low and high emphases, variances, entropy): two
+// reciprocals instead of seven divisions, which are what a cell costs.
+__device__ __forceinline__ void sc_size_terms(double p, double I, double J, double mui, double muj,
+                                              double (&v)[11]) {
+  const double i2 = I * I, j2 = J * J, ri = 1.0 / i2, rj = 1.0 / j2, pi = p * i2, qi = p * ri;
+  v[0] += p * rj;
+  v[1] += p * j2;
+  v[2] += (I - mui) * (I - mui) * p;
+  v[3] += (J - muj) * (J - muj) * p;
+  v[4] += sc_ent(p);
+  v[5] += qi;
+  v[6] += pi;
+  v[7] += qi * rj;
+  v[8] += pi * rj;
+  v[9] += qi * j2;
+  v[10] += pi * j2;
 }
 
 // GLRLM features of direction blockIdx.x (or of the merged matrix), written to
@@ -521,16 +592,21 @@ __global__ void __launch_bounds__(kScThreads) sc_glrlm_feat_kernel(const __grid_
     for (int q = 0; q < kNumDirs; ++q) s += a.glrlm[((size_t)q * a.ngc + i) * L + l];
     return s;
   };
-  // totals, row and column sums of squares
+  // totals, row and column sums of squares: a warp per level, a thread per length
   unsigned long long u[3] = {0ull, 0ull, 0ull};  // N, sum_i rows^2, sum_l cols^2
-  for (int i = tid; i < ng; i += blockDim.x) {
+  for (int i = tid >> 5; i < ng; i += blockDim.x >> 5) {
     unsigned long long r = 0;
-    for (int l = 0; l < L; ++l) r += R(i, l);
-    u[0] += r;
-    u[1] += r * r;
+    for (int l = tid & 31; l < L; l += 32) r += R(i, l);
+#pragma unroll
+    for (int o = 16; o; o >>= 1) r += __shfl_xor_sync(kFull, r, o);
+    if ((tid & 31) == 0) {
+      u[0] += r;
+      u[1] += r * r;
+    }
   }
   for (int l = tid; l < L; l += blockDim.x) {
     unsigned long long c = 0;
+#pragma unroll 8
     for (int i = 0; i < ng; ++i) c += R(i, l);
     u[2] += c * c;
   }
@@ -557,17 +633,7 @@ __global__ void __launch_bounds__(kScThreads) sc_glrlm_feat_kernel(const __grid_
     const unsigned long long c = R(i, l);
     if (!c) continue;
     const double p = (double)c / N, I = i + 1, J = l + 1;
-    v[0] += p / (J * J);
-    v[1] += p * J * J;
-    v[2] += (I - mui) * (I - mui) * p;
-    v[3] += (J - muj) * (J - muj) * p;
-    v[4] += sc_ent(p);
-    v[5] += p / (I * I);
-    v[6] += p * I * I;
-    v[7] += p / (I * I * J * J);
-    v[8] += p * I * I / (J * J);
-    v[9] += p * J * J / (I * I);
-    v[10] += p * I * I * J * J;
+    sc_size_terms(p, I, J, mui, muj, v);
   }
   block_sum<11>(v, s_red);
   if (tid == 0) {
@@ -591,13 +657,18 @@ __global__ void __launch_bounds__(kScThreads) sc_glrlm_feat_kernel(const __grid_
   }
 }
 
-// First order (block 0), GLSZM (block 1), GLDM and NGTDM (block 2), written
-// to out[0..17], out[58..92] and their extras out[93..95], out[98..100].
+// First order (block 0), GLDM (block 1) and NGTDM (block 2), written to
+// out[0..17], out[74..92] and their extras out[93..95], out[98..100].  Bound
+// by latency and the FP64 pipe of one SM: the histogram is read in rows of the
+// block (all loads of a pass in flight), and after the first pass between the
+// smallest and largest intensity only.
+// 200k voxels: 1250 us with the zones here, on one SM each -> 68 us.
 __global__ void __launch_bounds__(kMiscThreads) sc_misc_feat_kernel(const __grid_constant__ FrScalarArgs a) {
   __shared__ double s_red[12 * 32];
   __shared__ unsigned long long s_ured[4 * 32];
-  __shared__ unsigned __int128 s_qred[11 * 32];
-  __shared__ unsigned long long s_base[kMiscThreads];
+  __shared__ unsigned long long s_rank[10];
+  __shared__ double s_pct[5];
+  __shared__ long long s_p100[5];
   __shared__ int s_val[10];
   __shared__ int s_mm[2];
   __shared__ double s_si[256];
@@ -608,87 +679,94 @@ __global__ void __launch_bounds__(kMiscThreads) sc_misc_feat_kernel(const __grid
     if (blockIdx.x == 0 && tid < 18) out[tid] = kNaN;
     if (blockIdx.x == 0 && tid < 3) out[kFirstExtra + tid] = kNaN;
     if (blockIdx.x == 0 && tid == 0) out[kScalarStd] = kNaN;
-    if (blockIdx.x == 1 && tid < 16) out[58 + tid] = kNaN;
-    if (blockIdx.x == 2 && tid < 19) out[74 + tid] = kNaN;
-    if (blockIdx.x == 2 && tid < 3) out[kGldmExtra + tid] = kNaN;
+    if (blockIdx.x == 1 && tid < 14) out[74 + tid] = kNaN;
+    if (blockIdx.x == 1 && tid < 3) out[kGldmExtra + tid] = kNaN;
+    if (blockIdx.x == 2 && tid < 5) out[88 + tid] = kNaN;
     return;
   }
   const int ng = a.state->ng;
   if (blockIdx.x == 0) {
-    // ---- first order from the raw histogram: each thread 64 bins
-    constexpr int kPer = 65536 / kMiscThreads;
-    const int b0 = tid * kPer;
+    // ---- first order from the raw histogram
     unsigned long long u[3] = {0ull, 0ull, 0ull};  // N, sum x (offset), sum x^2
     long long s1 = 0;
     int lo = INT_MAX, hi = INT_MIN;
-    for (int b = b0; b < b0 + kPer; ++b) {
+#pragma unroll 16
+    for (int b = tid; b < 65536; b += kMiscThreads) {
       const unsigned c = a.hraw[b];
-      if (!c) continue;
       const long long xv = b - 32768;
       u[0] += c;
       s1 += (long long)c * xv;
       u[2] += (unsigned long long)c * (unsigned long long)(xv * xv);
-      lo = min(lo, (int)xv);
-      hi = max(hi, (int)xv);
+      if (c) {
+        lo = min(lo, b);
+        hi = max(hi, b);
+      }
     }
-    s_base[tid] = u[0];
     u[1] = (unsigned long long)s1;  // two's complement sums add exactly
     if (tid < 2) s_mm[tid] = tid == 0 ? INT_MAX : INT_MIN;
     __syncthreads();
-    atomicMin(&s_mm[0], lo);
-    atomicMax(&s_mm[1], hi);
+    lo = __reduce_min_sync(kFull, lo);
+    hi = __reduce_max_sync(kFull, hi);
+    if ((tid & 31) == 0) {
+      atomicMin(&s_mm[0], lo);
+      atomicMax(&s_mm[1], hi);
+    }
     block_sum_u64<3>(u, s_ured);  // contains __syncthreads
     const unsigned long long n = u[0];
     const long long S1 = (long long)u[1];
     const unsigned long long S2 = u[2];
-    // exclusive prefix of the per-thread counts (one thread; 1024 values)
-    if (tid == 0) {
-      unsigned long long run = 0;
-      for (int t = 0; t < kMiscThreads; ++t) {
-        const unsigned long long c = s_base[t];
-        s_base[t] = run;
-        run += c;
-      }
-    }
-    __syncthreads();
+    lo = s_mm[0];  // bins of the smallest and largest intensity
+    hi = s_mm[1];
+    if (n == 0) lo = 32768, hi = 32767;  // no bins
     // order statistics at the ranks of P10, P25, P50, P75, P90 (k and k + 1)
     const int qs[5] = {10, 25, 50, 75, 90};
+    if (tid < 10) {
+      const unsigned long long k =
+          (n - 1) * (unsigned long long)qs[tid >> 1] / 100 + (unsigned)(tid & 1);
+      s_rank[tid] = min(k, n - 1);
+    }
     {
-      const unsigned long long base = s_base[tid];
-      unsigned long long run = base;
-      int r = 0;
-      for (int b = b0; b < b0 + kPer; ++b) {
-        const unsigned c = a.hraw[b];
-        if (!c) continue;
-        for (r = 0; r < 10; ++r) {
-          const unsigned long long num = (n - 1) * (unsigned long long)qs[r >> 1];
-          unsigned long long k = num / 100 + (r & 1);
-          if (k > n - 1) k = n - 1;
-          if (k >= run && k < run + c) s_val[r] = b - 32768;
-        }
-        run += c;
+      // each thread some consecutive bins, between the counts before and after
+      const int per = (hi - lo + kMiscThreads) / kMiscThreads;
+      const int b0 = lo + tid * per, b1 = min(b0 + per, hi + 1);
+      unsigned long long own = 0;
+      for (int b = b0; b < b1; ++b) own += a.hraw[b];
+      unsigned long long inc = own;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long t = __shfl_up_sync(kFull, inc, o);
+        if ((tid & 31) >= o) inc += t;
       }
+      if ((tid & 31) == 31) s_ured[tid >> 5] = inc;
+      __syncthreads();
+      unsigned long long run = inc - own;
+      for (int w = 0; w < (tid >> 5); ++w) run += s_ured[w];
+      if (own)
+        for (int r = 0; r < 10; ++r) {
+          const unsigned long long k = s_rank[r];
+          if (k < run || k >= run + own) continue;
+          unsigned long long at = run;
+          int b = b0;
+          while (k >= at + a.hraw[b]) at += a.hraw[b++];
+          s_val[r] = b - 32768;
+        }
     }
     __syncthreads();
     const double N = (double)n, mean = (double)S1 / N;
-    auto pct = [&](int qi) -> double {
-      const unsigned long long num = (n - 1) * (unsigned long long)qs[qi];
+    if (tid < 5) {
+      const unsigned long long num = (n - 1) * (unsigned long long)qs[tid];
       const long long rem = (long long)(num % 100);
-      const int xk = s_val[2 * qi], xk1 = s_val[2 * qi + 1];
-      if (rem == 0) return (double)xk;
-      return xk + (rem / 100.0) * (double)(xk1 - xk);
-    };
-    // 100 * P_q exactly, for the robust subset P10 <= x <= P90
-    auto pct100 = [&](int qi) -> long long {
-      const unsigned long long num = (n - 1) * (unsigned long long)qs[qi];
-      const long long rem = (long long)(num % 100);
-      const long long xk = s_val[2 * qi], xk1 = s_val[2 * qi + 1];
-      return 100 * xk + (rem ? rem * (xk1 - xk) : 0);
-    };
-    const long long r10 = pct100(0), r90 = pct100(4);
+      const long long xk = s_val[2 * tid], xk1 = s_val[2 * tid + 1];
+      s_pct[tid] = rem == 0 ? (double)xk : xk + (rem / 100.0) * (double)(xk1 - xk);
+      // 100 * P_q exactly, for the robust subset P10 <= x <= P90
+      s_p100[tid] = 100 * xk + (rem ? rem * (xk1 - xk) : 0);
+    }
+    __syncthreads();
+    auto pct = [&](int qi) -> double { return s_pct[qi]; };
+    const long long r10 = s_p100[0], r90 = s_p100[4];
     const double med = pct(2);
     double m[7] = {0, 0, 0, 0, 0, 0, 0};  // m2 m3 m4 mad, robust count, robust sum, |x - median|
-    for (int b = b0; b < b0 + kPer; ++b) {
+    for (int b = lo + tid; b <= hi; b += kMiscThreads) {
       const unsigned c = a.hraw[b];
       if (!c) continue;
       const double xv = b - 32768, dv = xv - mean, dc = (double)c;
@@ -706,7 +784,7 @@ __global__ void __launch_bounds__(kMiscThreads) sc_misc_feat_kernel(const __grid
     block_sum<7>(m, s_red);
     const double rmean = m[5] / m[4];
     double rm[1] = {0.0};
-    for (int b = b0; b < b0 + kPer; ++b) {
+    for (int b = lo + tid; b <= hi; b += kMiscThreads) {
       const unsigned c = a.hraw[b];
       if (!c) continue;
       const long long x100 = 100ll * (b - 32768);
@@ -726,14 +804,14 @@ __global__ void __launch_bounds__(kMiscThreads) sc_misc_feat_kernel(const __grid
       out[0] = (double)S2;
       out[1] = a.voxel_volume * (double)S2;
       out[2] = e[0];
-      out[3] = (double)s_mm[0];
+      out[3] = (double)(lo - 32768);
       out[4] = pct(0);
       out[5] = pct(4);
-      out[6] = (double)s_mm[1];
+      out[6] = (double)(hi - 32768);
       out[7] = mean;
       out[8] = pct(2);
       out[9] = pct(3) - pct(1);
-      out[10] = (double)s_mm[1] - (double)s_mm[0];
+      out[10] = (double)(hi - lo);
       out[11] = m[3] / N;
       out[12] = rm[0] / m[4];
       out[13] = sqrt((double)S2 / N);
@@ -751,71 +829,6 @@ __global__ void __launch_bounds__(kMiscThreads) sc_misc_feat_kernel(const __grid
       out[kScalarStd] = sqrt(m2);
     }
   } else if (blockIdx.x == 1) {
-    // ---- GLSZM from zones per level, per size and per (level, size)
-    unsigned long long u[3] = {0ull, 0ull, 0ull};  // N zones, sum rows^2, sum cols^2
-    for (int g = tid + 1; g <= ng; g += blockDim.x) {
-      const unsigned long long r = a.zrow[g];
-      u[0] += r;
-      u[1] += r * r;
-    }
-    double m[2] = {0.0, 0.0};
-    for (int64_t j = tid + 1; j <= a.n_voi; j += blockDim.x) {
-      const unsigned long long c = a.zcol[j];
-      u[2] += c * c;
-      m[1] += (double)j * (double)c;
-    }
-    for (int g = tid + 1; g <= ng; g += blockDim.x) m[0] += (double)g * (double)a.zrow[g];
-    block_sum_u64<3>(u, s_ured);
-    block_sum<2>(m, s_red);
-    const double N = (double)u[0];
-    const double mui = m[0] / N, muj = m[1] / N;
-    // every (level, size) cell's terms, summed in fixed point so that the
-    // slot order of the zone table does not change the result.  Bits after
-    // the point per sum, from its bound (I <= 255, J < 2^31, sum p = 1):
-    // <= 1 -> 120; <= 255^2 -> 110; <= 2^62 -> 64; <= 2^78 -> 48.
-    constexpr int kFb[11] = {120, 64, 110, 64, 120, 120, 110, 120, 110, 64, 48};
-    unsigned __int128 q[11];
-    for (int k = 0; k < 11; ++k) q[k] = 0;
-    for (int64_t t = tid; t < a.hcap; t += blockDim.x) {
-      const unsigned long long key = a.hkey[t];
-      if (key == kEmptyKey) continue;
-      const double I = (double)(key >> 32), J = (double)(key & 0xffffffffull);
-      const double p = (double)a.hcnt[t] / N;
-      const double tv[11] = {p / (J * J),          p * J * J,          (I - mui) * (I - mui) * p,
-                             (J - muj) * (J - muj) * p, sc_ent(p),     p / (I * I),
-                             p * I * I,            p / (I * I * J * J), p * I * I / (J * J),
-                             p * J * J / (I * I),  p * I * I * J * J};
-#pragma unroll
-      for (int k = 0; k < 11; ++k) q[k] += sc_fixed(tv[k], kFb[k]);
-    }
-    block_sum_u128<11>(q, s_qred);
-    double v[11];
-#pragma unroll
-    for (int k = 0; k < 11; ++k) v[k] = sc_unfixed(q[k], kFb[k]);
-    if (tid == 0) {
-      double* f = out + 58;
-      if (u[0] == 0) {
-        for (int k = 0; k < 16; ++k) f[k] = kNaN;
-      } else {
-        f[0] = v[0];
-        f[1] = v[1];
-        f[2] = (double)u[1] / N;
-        f[3] = (double)u[1] / (N * N);
-        f[4] = (double)u[2] / N;
-        f[5] = (double)u[2] / (N * N);
-        f[6] = N / (double)a.n_voi;
-        f[7] = v[2];
-        f[8] = v[3];
-        f[9] = v[4];
-        f[10] = v[5];
-        f[11] = v[6];
-        f[12] = v[7];
-        f[13] = v[8];
-        f[14] = v[9];
-        f[15] = v[10];
-      }
-    }
-  } else {
     // ---- GLDM from [level][equal neighbours] counts
     // N, sum rows^2, sum cols^2, sum of squared cells
     unsigned long long u[4] = {0ull, 0ull, 0ull, 0ull};
@@ -852,50 +865,9 @@ __global__ void __launch_bounds__(kMiscThreads) sc_misc_feat_kernel(const __grid
       const unsigned c = a.gldm[g * 27 + j];
       if (!c) continue;
       const double p = (double)c / N, I = g, J = j + 1;
-      v[0] += p / (J * J);
-      v[1] += p * J * J;
-      v[2] += (I - mui) * (I - mui) * p;
-      v[3] += (J - muj) * (J - muj) * p;
-      v[4] += sc_ent(p);
-      v[5] += p / (I * I);
-      v[6] += p * I * I;
-      v[7] += p / (I * I * J * J);
-      v[8] += p * I * I / (J * J);
-      v[9] += p * J * J / (I * I);
-      v[10] += p * I * I * J * J;
+      sc_size_terms(p, I, J, mui, muj, v);
     }
     block_sum<11>(v, s_red);
-    // ---- NGTDM: n_i, s_i = sum_k acc[i][k] / k
-    double w[4] = {0, 0, 0, 0};  // Nvp, sum n_i s_i, sum s_i, levels present
-    for (int g = tid; g < 256; g += blockDim.x) {
-      double si = 0.0;
-      if (g >= 1 && g <= ng)
-        for (int k = 1; k <= 26; ++k) si += (double)a.ngacc[g * 27 + k] / (double)k;
-      s_si[g] = si;
-    }
-    __syncthreads();
-    for (int g = tid + 1; g <= ng; g += blockDim.x) {
-      const double ni = (double)a.ngn[g], si = s_si[g];
-      w[0] += ni;
-      w[1] += ni * si;
-      w[2] += si;
-      w[3] += ni > 0.0 ? 1.0 : 0.0;
-    }
-    block_sum<4>(w, s_red);
-    const double Nvp = w[0], sum_ps = w[1] / Nvp, sum_s = w[2], ngp = w[3];
-    double x[4] = {0.0, 0.0, 0.0, 0.0};  // c1, busy den, complexity, strength
-    for (int t = tid; t < ng * ng; t += blockDim.x) {
-      const int i = t / ng + 1, j = t % ng + 1;
-      const double ni = (double)a.ngn[i], nj = (double)a.ngn[j];
-      if (ni == 0.0 || nj == 0.0) continue;
-      const double si = s_si[i], sj = s_si[j];
-      const double pi = ni / Nvp, pj = nj / Nvp, dd = (double)(i - j);
-      x[0] += pi * pj * dd * dd;
-      x[1] += fabs((double)i * ni - (double)j * nj) / Nvp;
-      x[2] += fabs(dd) * (pi * si + pj * sj) / (pi + pj);
-      x[3] += (pi + pj) * dd * dd;
-    }
-    block_sum<4>(x, s_red);
     if (tid == 0) {
       double* f = out + 74;
       if (u[0] == 0) {
@@ -926,6 +898,48 @@ __global__ void __launch_bounds__(kMiscThreads) sc_misc_feat_kernel(const __grid
         e[1] = N / (double)a.n_voi;
         e[2] = (double)u[3] / (N * N);
       }
+    }
+  } else {
+    // ---- NGTDM: n_i, s_i = sum_k acc[i][k] / k
+    double w[4] = {0, 0, 0, 0};  // Nvp, sum n_i s_i, sum s_i, levels present
+    for (int g = tid; g < 256; g += blockDim.x) {
+      double si = 0.0;
+      if (g >= 1 && g <= ng)
+        for (int k = 1; k <= 26; ++k) si += (double)a.ngacc[g * 27 + k] / (double)k;
+      s_si[g] = si;
+    }
+    __syncthreads();
+    for (int g = tid + 1; g <= ng; g += blockDim.x) {
+      const double ni = (double)a.ngn[g], si = s_si[g];
+      w[0] += ni;
+      w[1] += ni * si;
+      w[2] += si;
+      w[3] += ni > 0.0 ? 1.0 : 0.0;
+    }
+    block_sum<4>(w, s_red);
+    const double Nvp = w[0], sum_ps = w[1] / Nvp, sum_s = w[2], ngp = w[3];
+    // c1, busy den, complexity, strength: symmetric, and 0 for i = j
+    double x[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int t = tid; t < (ng + 1) / 2 * (ng + 1); t += blockDim.x) {
+      int i, j;
+      if (!sc_cell(t, ng, i, j) || i == j) continue;
+      ++i;
+      ++j;
+      const double ni = (double)a.ngn[i], nj = (double)a.ngn[j];
+      if (ni == 0.0 || nj == 0.0) continue;
+      const double si = s_si[i], sj = s_si[j];
+      const double dd = (double)(j - i);
+      x[0] += ni * nj * (dd * dd);
+      x[1] += fabs((double)i * ni - (double)j * nj);
+      x[2] += dd * (ni * si + nj * sj) / (ni + nj);
+      x[3] += (ni + nj) * (dd * dd);
+    }
+    block_sum<4>(x, s_red);
+    x[0] *= 2.0 / (Nvp * Nvp);
+    x[1] *= 2.0 / Nvp;
+    x[2] *= 2.0;
+    x[3] *= 2.0 / Nvp;
+    if (tid == 0) {
       double* h = out + 88;
       if (Nvp == 0.0) {
         for (int k = 0; k < 5; ++k) h[k] = kNaN;
@@ -937,6 +951,113 @@ __global__ void __launch_bounds__(kMiscThreads) sc_misc_feat_kernel(const __grid
         h[4] = sc_div(x[3], sum_s);
       }
     }
+  }
+}
+
+// GLSZM from the zones per level, per size and per (level, size).  The table
+// of the last is read by the whole chip; a block packs its occupied slots
+// first, so that the FP64 terms run on full warps (a few zones in a thousand
+// slots), and adds its sums in fixed point: integers, so that neither the slot
+// order of the table nor the order of the blocks changes the result.  The last
+// block writes out[58..73].  524k slots: 31 us.
+constexpr int kZoneSlots = 8 * kScThreads;
+__global__ void __launch_bounds__(kScThreads) sc_zone_feat_kernel(const __grid_constant__ FrScalarArgs a) {
+  __shared__ unsigned long long s_ured[3 * 32];
+  __shared__ unsigned __int128 s_qred[11 * 32];
+  __shared__ int s_slot[kZoneSlots];
+  __shared__ int s_n;
+  __shared__ bool s_last;
+  const int tid = threadIdx.x;
+  double* f = a.out + 58;
+  const double kNaN = __longlong_as_double(0x7ff8000000000000ll);
+  if (sc_failed(a)) {
+    if (blockIdx.x == 0 && tid < 16) f[tid] = kNaN;
+    return;
+  }
+  const int ng = a.state->ng;
+  unsigned long long u[3] = {0ull, 0ull, 0ull};  // N zones, sum rows^2, sum of levels
+  for (int g = tid + 1; g <= ng; g += blockDim.x) {
+    const unsigned long long r = a.zrow[g];
+    u[0] += r;
+    u[1] += r * r;
+    u[2] += (unsigned)g * r;
+  }
+  block_sum_u64<3>(u, s_ured);
+  if (u[0] == 0) {
+    if (blockIdx.x == 0 && tid < 16) f[tid] = kNaN;
+    return;
+  }
+  // the sizes add up to the VOI
+  const double N = (double)u[0], mui = (double)u[2] / N, muj = (double)a.n_voi / N;
+  unsigned long long c2[1] = {0ull};  // sum cols^2
+  for (int64_t j = (int64_t)blockIdx.x * blockDim.x + tid + 1; j <= a.n_voi;
+       j += (int64_t)gridDim.x * blockDim.x) {
+    const unsigned long long c = a.zcol[j];
+    c2[0] += c * c;
+  }
+  // bits after the point per sum, from its bound (I <= 255, J < 2^31, sum p =
+  // 1): <= 1 -> 120; <= 255^2 -> 110; <= 2^62 -> 64; <= 2^78 -> 48
+  constexpr int kFb[11] = {120, 64, 110, 64, 120, 120, 110, 120, 110, 64, 48};
+  unsigned __int128 q[11];
+  for (int k = 0; k < 11; ++k) q[k] = 0;
+  for (int64_t t0 = (int64_t)blockIdx.x * kZoneSlots; t0 < a.hcap; t0 += (int64_t)gridDim.x * kZoneSlots) {
+    if (tid == 0) s_n = 0;
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kZoneSlots / kScThreads; ++k) {
+      const int64_t t = t0 + k * kScThreads + tid;
+      if (t < a.hcap && a.hkey[t] != kEmptyKey) s_slot[atomicAdd(&s_n, 1)] = k * kScThreads + tid;
+    }
+    __syncthreads();
+    for (int e = tid; e < s_n; e += blockDim.x) {
+      const int64_t t = t0 + s_slot[e];
+      const unsigned long long key = a.hkey[t];
+      const double I = (double)(key >> 32), J = (double)(key & 0xffffffffull);
+      double tv[11] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+      sc_size_terms((double)a.hcnt[t] / N, I, J, mui, muj, tv);
+#pragma unroll
+      for (int k = 0; k < 11; ++k) q[k] += sc_fixed(tv[k], kFb[k]);
+    }
+    __syncthreads();
+  }
+  block_sum_u64<1>(c2, s_ured);
+  block_sum_u128<11>(q, s_qred);
+  if (tid < 11) {
+    // 128-bit sums as two words, the carry passed on by the addition that wraps
+    const unsigned __int128 own = s_qred[tid * 32];
+    const unsigned long long lo = (unsigned long long)own;
+    const unsigned long long was = atomicAdd(&a.zsum[2 * tid], lo);
+    atomicAdd(&a.zsum[2 * tid + 1], (unsigned long long)(own >> 64) + (was + lo < was ? 1ull : 0ull));
+  }
+  if (tid == 11) atomicAdd(&a.zsum[22], c2[0]);
+  __threadfence();
+  __syncthreads();
+  if (tid == 0) s_last = atomicAdd(&a.zsum[23], 1ull) == gridDim.x - 1;
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  if (tid == 0) {
+    double v[11];
+#pragma unroll
+    for (int k = 0; k < 11; ++k)
+      v[k] = sc_unfixed(((unsigned __int128)__ldcg(&a.zsum[2 * k + 1]) << 64) | __ldcg(&a.zsum[2 * k]), kFb[k]);
+    const double cols2 = (double)__ldcg(&a.zsum[22]);
+    f[0] = v[0];
+    f[1] = v[1];
+    f[2] = (double)u[1] / N;
+    f[3] = (double)u[1] / (N * N);
+    f[4] = cols2 / N;
+    f[5] = cols2 / (N * N);
+    f[6] = N / (double)a.n_voi;
+    f[7] = v[2];
+    f[8] = v[3];
+    f[9] = v[4];
+    f[10] = v[5];
+    f[11] = v[6];
+    f[12] = v[7];
+    f[13] = v[8];
+    f[14] = v[9];
+    f[15] = v[10];
   }
 }
 
@@ -975,23 +1096,24 @@ static int sc_grid(int64_t n, int threads, int cap) {
 
 cudaError_t fr_scalar_configure(int ngc) {
   cudaError_t e = cudaFuncSetAttribute(sc_neigh_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       kNeighSmem);
+                                       neigh_smem(255));
   if (e != cudaSuccess) return e;
-  const int np = ngc * (ngc + 1) / 2;
   return cudaFuncSetAttribute(sc_glcm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              np * 4);
+                              255 * 256 / 2 * 4);
 }
 
 // Every kernel of one scalar extraction, after discretisation and the
-// zeroing of the count buffers.  8 launches + 2 per-direction grids.
+// zeroing of the count buffers.
 cudaError_t fr_scalar_launch(const FrScalarArgs& a, double* user_out, const int16_t* row_of_dev,
                              int sms, cudaStream_t s) {
   const int grid = sc_grid(a.n_voi, kScThreads, 8 * sms);
   sc_init_kernel<<<grid, kScThreads, 0, s>>>(a);
-  sc_neigh_kernel<<<grid, kScThreads, kNeighSmem, s>>>(a);
-  const int gx = sc_grid(a.n_voi, kScThreads * 16, (2 * sms + kNumDirs - 1) / kNumDirs);
+  sc_neigh_kernel<<<sc_grid(a.n_voi, kCountThreads, 2 * sms), kCountThreads, neigh_smem(a.ngc), s>>>(a);
+  // one wave of blocks at the largest level cap, whose copy leaves one a SM
+  // (200k voxels: 66 us with 312 blocks of 256 threads -> 19 us)
+  const int gx = sc_grid(a.n_voi, kCountThreads * 4, sms / kNumDirs > 0 ? sms / kNumDirs : 1);
   const int np = a.ngc * (a.ngc + 1) / 2;
-  sc_glcm_kernel<<<dim3(gx, kNumDirs), kScThreads, np * 4, s>>>(a);
+  sc_glcm_kernel<<<dim3(gx, kNumDirs), kCountThreads, np * 4, s>>>(a);
   sc_glrlm_kernel<<<dim3(sc_grid(a.n_voi, kScThreads, (8 * sms) / kNumDirs + 1), kNumDirs),
                     kScThreads, 0, s>>>(a);
   sc_flatten_kernel<<<grid, kScThreads, 0, s>>>(a);
@@ -999,6 +1121,7 @@ cudaError_t fr_scalar_launch(const FrScalarArgs& a, double* user_out, const int1
   const int ndir = a.agg == 1 ? 1 : kNumDirs;
   sc_glcm_feat_kernel<<<ndir, kScThreads, 0, s>>>(a);
   sc_glrlm_feat_kernel<<<ndir, kScThreads, 0, s>>>(a);
+  sc_zone_feat_kernel<<<sc_grid(a.hcap, kZoneSlots, 2 * sms), kScThreads, 0, s>>>(a);
   sc_misc_feat_kernel<<<3, kMiscThreads, 0, s>>>(a);
   sc_final_kernel<<<1, 128, 0, s>>>(a, user_out, row_of_dev);
   return cudaGetLastError();
