@@ -109,3 +109,9 @@ def test_side_seven(n):
 @pytest.mark.parametrize("n", [4, 5, 7, 8, 9, 10, 11, 12, 13, 14, 15, 16])
 def test_up_to_sixteen_rows(n, loops, merged):
     _check(n, loops, 4, aggregation=merged)
+
+
+@pytest.mark.parametrize("loops", [0, 1])
+@pytest.mark.parametrize("n", [17, 18, 19, 20, 21, 22, 23, 24])
+def test_seventeen_rows_and_more(n, loops):
+    _check(n, loops, 6)
