@@ -147,7 +147,7 @@ struct FrMapArgs {
   int32_t slab_ngc;    // level cap the slab is laid out for
   FrArena arena;
   float* fb;           // per-warp matrices of many-level MCC solves (kNumDirs x
-  int64_t fb_stride;   // kFbDir floats each) handed to the CTA's pool; null: inline
+  int64_t fb_stride;   // kFbDir floats each) handed to the CTA's pool
   int32_t* dbg;        // debug records (DUMP kernel only)
   int64_t dbg_stride;  // int32 per record
   int64_t timeout_ns;  // bound of every device wait

@@ -189,13 +189,11 @@ __device__ __forceinline__ void map_voxel(const FrMapArgs& args, const FrJob& jo
   consumer_bar(nt);
   if (refill && threadIdx.x == 0) feed(args, fd, stage, parity);
   if (job.families & kFamGLCM) {
-    const bool use_pool = args.fb != nullptr && (job.families & kFamMCC) != 0;
-    const float* fb = args.fb + (size_t)blockIdx.x * args.consumer_warps * args.fb_stride;
-    if (work)
-      vox_glcm<DUMP>(off, job, d_glcm, pool_off,
-                     use_pool ? (float*)fb + (threadIdx.x >> 5) * args.fb_stride : nullptr);
-    if (work && use_pool) pool_list_slots(pool_off, off);
-    if (use_pool) {
+    const bool mcc = (job.families & kFamMCC) != 0;
+    float* fb = args.fb + (size_t)blockIdx.x * args.consumer_warps * args.fb_stride;
+    if (work) vox_glcm<DUMP>(off, job, d_glcm, pool_off, fb + (threadIdx.x >> 5) * args.fb_stride);
+    if (work && mcc) pool_list_slots(pool_off, off);
+    if (mcc) {
       consumer_bar(nt);  // the task list is complete
       const volatile int* pc = (const volatile int*)(fr_smem + pool_off);
       if (pc[0] + pc[1] + pc[2] + pc[3] + pc[4] > 0) {
