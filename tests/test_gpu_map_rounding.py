@@ -21,6 +21,8 @@ pytestmark = pytest.mark.gpu
 NAMES = {n: i for i, n in enumerate(O.feature_names())}
 GLCM = {"glcm_ClusterTendency": 6, "glcm_DifferenceVariance": 6, "glcm_JointEnergy": 6,
         "glcm_SumSquares": 6, "glcm_SumVariance": 6, "glcm_ClusterProminence": 8}
+GLRLM = {"glrlm_GrayLevelNonUniformityNormalized": 6, "glrlm_RunLengthNonUniformityNormalized": 6,
+         "glrlm_GrayLevelVariance": 6, "glrlm_RunVariance": 6}
 
 
 def _distances(names, shape, r, **kw):
@@ -46,8 +48,16 @@ def _check(names, shape, r, **kw):
     assert not bad, bad
 
 
-@pytest.mark.parametrize("r, disc", [(1, dict(disc_mode=1, bin_width=25.0)),
-                                     (2, dict(disc_mode=1, bin_width=25.0)),
-                                     (3, dict(disc_mode=0, bin_count=64))])
+WINDOWS = pytest.mark.parametrize("r, disc", [(1, dict(disc_mode=1, bin_width=25.0)),
+                                              (2, dict(disc_mode=1, bin_width=25.0)),
+                                              (3, dict(disc_mode=0, bin_count=64))])
+
+
+@WINDOWS
 def test_glcm(r, disc):
     _check(GLCM, (20, 24, 28), r, **disc)
+
+
+@WINDOWS
+def test_glrlm(r, disc):
+    _check(GLRLM, (20, 24, 28), r, **disc)
