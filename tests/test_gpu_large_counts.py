@@ -43,3 +43,23 @@ def test_merged(r, nlev):
 @pytest.mark.parametrize("nlev", [2, 16, 64])
 def test_side_fifteen(nlev, fill):
     _check(7, nlev, nlev, fill)
+
+
+@pytest.mark.parametrize("kw", [dict(), dict(glcm_distance=2), dict(aggregation=1)])
+@pytest.mark.parametrize("share", [0.21, 0.5, 0.98])
+@pytest.mark.parametrize("r", [3, 7])
+def test_widest_span(r, share, kw):
+    # two levels 254 apart (and a few between): the largest power sums and
+    # third moments of the class sums (a share of 0.21 has the largest)
+    rng = np.random.default_rng(r)
+    shape = (2 * r + 1, 2 * r + 2, 2 * r + 3)
+    img = np.where(rng.random(shape) < share, 254, 0)
+    img = np.where(rng.random(shape) < 0.02, rng.integers(0, 255, shape), img).astype(np.int16)
+    img.flat[0], img.flat[1] = 0, 254
+    kw = dict(disc_mode=0, bin_count=255, kernel_radius=r, **kw)
+    voxels = np.unique(np.append(rng.choice(img.size, 24, replace=False),
+                                 (r * shape[1] + r) * shape[2] + r)).astype(np.int64)
+    mask = np.ones(shape, np.uint8)
+    got, _, feats = H.gpu_map(img, mask, features=ALL, **kw)
+    ref, _, _, _ = H.oracle_map(img, mask, voxels=voxels, **kw)
+    parity.assert_close(got[:, voxels], ref[feats], [O.feature_names()[f] for f in feats])
