@@ -40,10 +40,10 @@ constexpr int kMaxConsumerWarps = 16;
 constexpr int kPadBytes = (7 + 2) * (7 + 2) * 8;
 constexpr int kMaxStages = 4;
 // CTA pool of MCC solves: at most one per direction per warp; with more than
-// kCapL levels a direction's S - u u^T is the packed upper triangle of its m x
-// m matrix (m (m + 1) / 2 contiguous floats, each written once) in the warp's
-// global scratch (kFbDir floats per direction).  kFbWords: 32-bit words of the
-// pool's counters (12) and lists.
+// kCapL levels a direction's m x m matrix S - u u^T lies in the warp's global
+// scratch (kFbDir floats per direction), square with rows of 16 up to 16 levels,
+// else as the packed upper triangle (m (m + 1) / 2 contiguous floats).
+// kFbWords: 32-bit words of the pool's counters (12) and lists.
 constexpr int kFbTasks = kMaxConsumerWarps * kNumDirs;
 constexpr int kFbWords = 12 + kFbTasks + 3 * kFbTasks / 2;
 constexpr int kFbDir = kMCap * kMCap;
@@ -189,7 +189,9 @@ struct FrScalarArgs {
 
 // Big-region layout for caps (mc, bc) and window size w.
 struct BigLayout {
-  int32_t cnt, marg, prank, sbin, dbin, vec;  // GLCM (vec: 4 float vectors of mc)
+  int32_t cnt, marg, prank, sbin, dbin, vec;  // GLCM (vec: the end of the dense path's
+                                              // counts; the tables of the other two
+                                              // paths go on to slots)
   int32_t slots;                              // GLCM MCC: the directions' matrices
   int32_t csn, cst;                           // GLCM ClusterShade numerators (f64), totals
   int32_t rhist, rlv, rlen;                  // GLRLM

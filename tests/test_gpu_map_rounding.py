@@ -4,7 +4,7 @@ A feature that is an exact integer over a power of a direction's total is
 rounded a known number of times.  Independent roundings to nearest of a value
 with mantissa 1 have a relative rms of 2^-24 / sqrt(3) each, so k of them at most
 sqrt(k) times that over a map (2-norm of the difference over 2-norm of the map).
-k counts the numerator, the reciprocal of the total's power, the product, the
+k counts at most the numerator, the reciprocal of the total's power, the product, the
 sum over directions, and two for the division by their number; a numerator of
 128 bits is rounded twice, and T^4 itself once."""
 import math
